@@ -97,7 +97,9 @@ typedef struct {
                              and residual in a first pass, X^T R in a second; up to 64 coefficient
                              columns per launch, no tile options): CUDA cores, or, FP32 X of some
                              size, tensor cores (X and the coefficients split into three BF16
-                             terms each, FP32 sums; up to 80 columns per launch).  Auto: FP32 / FP64
+                             terms each, which hold all their bits, compensated FP32 sums:
+                             no further from 64 bits than the CUDA cores; up to 64 columns
+                             per launch).  Auto: FP32 / FP64
                              storage on
                              engine 1, or on engine 4 where no engine-1 tile fits (wide problems with
                              many classes: FP32 X with K - 1 > 12 and p > 10240), K - 1 exceeds

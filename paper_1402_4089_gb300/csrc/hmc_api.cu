@@ -374,23 +374,27 @@ hmc_status choose_tc(hmc_ctx* h, Problem& P, bool* ok) {
 }
 
 // Whether both passes of an FP32 problem go to the tensor cores (lpg_split.cu).
-// They cost about the same for any C <= 16 (X streamed twice, split on chip: n=1e4
-// p=5000 80 us for C = 4, 82 for C = 14) and little more up to C = 80, while the CUDA-core
-// engines grow with C; against that stand six launches instead of three (about 10 us).
-// Measured over n in 20 .. 1e5, p in 10 .. 2e4 (us per gradient, CUDA cores -> tensor
-// cores; the lines where they lose were measured with a form of the passes about 10 us
-// slower):
-//   C >= 32: n=300 p=300 C=36 48 -> 31; n=1e4 p=2e4 C=76 4508 -> 347.  Wide X with
-//     few rows loses: n=100 p=5000 C=38 54 -> 73.
-//   C 19 .. 31: n=300 p=128 39 -> 29, n=1e4 p=785 90 -> 43, n=1000 p=785 48 -> 31, but
-//     n=1000 p=300 31 -> 33, n=300 p=5000 40 -> 50.
-//   C 10 .. 18: n=1e4 p=5000 C=14 205 -> 82; n=3000 p=2000 C=11 43 -> 37, but
+// They cost about the same for any C <= 32 (X streamed twice, split on chip: n=1e4
+// p=5000 89 us for C = 4, 91 for C = 14) and half as much again up to C = 64, while the
+// CUDA-core engines grow with C; against that stand six launches instead of three (about
+// 10 us).  Measured over n in 20 .. 2e6, p in 4 .. 2e4 (us per gradient, CUDA cores ->
+// tensor cores; the lines where they lose were measured with a form of the passes that
+// took about as long):
+//   C >= 32: n=300 p=300 C=36 56 -> 34; n=1e4 p=2e4 C=76 4511 -> 863; n=60 p=1000 C=39
+//     39.6 -> 39.5.  Wide X with few rows loses: n=100 p=5000 C=38 54 -> 73.
+//   C 19 .. 31: n=1e4 p=785 91 -> 44, n=1000 p=785 48 -> 31, but n=1000 p=300 31 -> 33,
+//     n=300 p=5000 40 -> 50.
+//   C 10 .. 18: n=1e4 p=5000 C=14 205 -> 91; n=3000 p=2000 C=11 44 -> 39, but
 //     n=1000 p=2000 C=14 31 -> 38.
-//   C 7 .. 9: n=6e4 p=785 139 -> 85, n=1e4 p=300 42 -> 33, n=1000 p=2e4 C=9 86 -> 54;
-//     n=3000 p=2000 37 -> 42.
-//   C < 7: the fused pass reads X once and stays (n=1e4 p=5000 C=4 80.5 -> 80.3).
+//   C 7 .. 9: n=6e4 p=785 142 -> 93, n=1e4 p=300 44 -> 35, n=2e4 p=4 C=7 32 -> 29, n=1000
+//     p=2e4 C=9 87 -> 58; n=3000 p=2000 37 -> 42.
+//   C < 7: the fused pass reads X once and stays (n=1e4 p=5000 C=4 80.5 -> 80.3 when the
+//     passes were some 8% faster).
+// A call with fewer chains than max_chains is no slower than on the engine it had (one
+// chain of eight, n=1e4 p=785 K=4 42 -> 36, n=1000 p=2000 K=10 42 -> 34; one of 64, n=1e4
+// p=300 K=2 40 -> 31).
 // `two`: the choice is between the two-pass engines only (engine 4 on request, or no
-// fused tile), whose CUDA-core form costs more: n=1e4 p=5000 C=9 183 -> 82.
+// fused tile), whose CUDA-core form costs more: n=1e4 p=5000 C=9 185 -> 90.
 bool split_pays(int64_t n, int64_t p, int64_t c_all, bool two) {
   if (c_all >= 32) return p <= 1000 || n >= 1000 || p <= 8 * n;
   if (c_all >= 19) return n >= 2000 || p <= 200 || (n >= 700 && p >= 700);

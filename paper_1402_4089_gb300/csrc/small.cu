@@ -55,11 +55,11 @@ __device__ __forceinline__ double prior_term(ST b, int kind, double s) {
     return -(x * x) / (2.0 * s * s);
   }
 }
-// s2 = s * s, inv = 1 / (s * s) (an FP64 division takes as long as the dot products of a row).
+// s2 = s * s.
 template <typename ST>
-__device__ __forceinline__ ST prior_deriv(ST b, int kind, ST s2, ST inv) {
+__device__ __forceinline__ ST prior_deriv(ST b, int kind, ST s2) {
   if (kind == HMC_PRIOR_CAUCHY) return ST(-2.0) * b / (s2 + b * b);
-  return sizeof(ST) == 8 ? -b * inv : -b / s2;
+  return -b / s2;
 }
 
 __device__ __forceinline__ void st_peer(uint32_t addr, float v) {
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const SmallArgs A) {
     w.item = t - w.blk * items;
     return w;
   };
-  const AT s2 = AT(A.prior_scale * A.prior_scale), inv_s2 = AT(1.0 / (A.prior_scale * A.prior_scale));
+  const AT s2 = AT(A.prior_scale * A.prior_scale);
   const int cblk = (C + kCB - 1) / kCB;
   const Walk wz = walk(cblk * rows, rows), wg = walk(cblk * p, p);
   int rw = 32;                     // threads that take a row each, a power of two
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_kernel(const SmallArgs A) {
       if (h < S)
 #pragma unroll
         for (int s = 0; s < 16; s += 2 * h) v[s] += v[s + h];
-    return v[0] + prior_deriv(beta[e0 + e], A.prior_kind, s2, inv_s2);
+    return v[0] + prior_deriv(beta[e0 + e], A.prior_kind, s2);
   };
   auto set_beta = [&](int e, AT v) {       // owned coefficient e, in every CTA
     AT* d = beta + e0 + e;

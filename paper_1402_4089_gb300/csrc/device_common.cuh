@@ -140,6 +140,14 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 blo
   return cudaLaunchKernelEx(&cfg, kernel, Params(given)...);
 }
 
+// ------------------------------------------------------------ exact sums
+// Knuth's two-sum: a + b rounded, and what the rounding lost.
+__device__ __forceinline__ float two_sum(float a, float b, float& lost) {
+  const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
+  lost = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  return s;
+}
+
 // ------------------------------------------------------------ bulk copies
 // Contiguous global -> shared copy completing on a local mbarrier
 // (both addresses 16-byte aligned, bytes a multiple of 16).

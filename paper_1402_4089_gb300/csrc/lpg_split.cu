@@ -811,9 +811,10 @@ __global__ void __launch_bounds__(128) predict_prob_kernel(float* __restrict__ z
 
 // FP64 sums of the probabilities in draw order: block 32 rows x K classes, one thread
 // per (row, class), kFlight draws in flight.  Their FP32 probabilities are summed with
-// their rounding errors carried (Knuth's two-sum; 2^-47 of the sum is dropped) before
-// they meet the FP64 sum: bound by the FP64 units, n=1e4 K=10 and 100 draws took
-// 68 us with a conversion and an addition for each, 28 us so.  `first`: the sums start at zero, else at
+// their rounding errors and theirs carried (two-sum, twice; 2^-71 of the sum is dropped)
+// before they meet the FP64 sum, which rounds three times where it rounded eight: bound by
+// the FP64 units, n=1e4 K=10 and 100 draws took 68 us with a conversion and an addition for
+// each, 28 us with the first errors alone (the call takes no longer with both).  `first`: the sums start at zero, else at
 // `acc`; total_draws > 0 (last launch): the means and their argmax (lowest class on a
 // tie) are written, else the sums go to `acc`.
 __global__ void predict_sum_kernel(const float* __restrict__ zpart, int64_t ntiles, int32_t N, int64_t n, int64_t ndraws,
@@ -844,14 +845,14 @@ __global__ void predict_sum_kernel(const float* __restrict__ zpart, int64_t ntil
           }
         }
       }
-      float hi = v[0], lo = 0.f;
+      float hi = v[0], lo = 0.f, rest = 0.f;
 #pragma unroll
       for (int i = 1; i < kFlight; ++i) {
-        const float t = __fadd_rn(hi, v[i]), w = __fsub_rn(t, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, w)), __fsub_rn(v[i], w)));
-        hi = t;
+        hi = two_sum(hi, v[i], v[i]);
+        lo = two_sum(lo, v[i], v[i]);
+        rest = __fadd_rn(rest, v[i]);
       }
-      s += double(hi) + double(lo);
+      s += (double(hi) + double(lo)) + double(rest);
     }
     if (total_draws == 0.0) {
       acc[size_t(row) * K + k] = s;

@@ -36,20 +36,21 @@ __device__ __forceinline__ double prior_term(ST b, int kind, double s) {
 }
 
 // The FP32 prior terms of four coefficients as one FP64 value: summed in FP32 with the
-// rounding errors carried along (Knuth's two-sum; what is dropped is 2^-48 of the sum),
-// so that FP64 units see two conversions and one addition, not four of each.
+// rounding errors and theirs carried along (Knuth's two-sum, twice; what is dropped is
+// 2^-72 of the sum), so that FP64 units see three conversions and two additions, not
+// four of each, and round twice.
 __device__ __forceinline__ double prior_quad(const float4 b, int kind, float sc) {
-  const float t[4] = {prior_term32(b.x, kind, sc), prior_term32(b.y, kind, sc), prior_term32(b.z, kind, sc),
-                      prior_term32(b.w, kind, sc)};
-  float s = t[0], e = 0.f;
+  auto term = [&](int i) { return prior_term32(i == 0 ? b.x : i == 1 ? b.y : i == 2 ? b.z : b.w, kind, sc); };
+  float t[4] = {term(0), term(1), term(2), term(3)};
+  float s = t[0], e = 0.f, e2 = 0.f;
 #pragma unroll
   for (int i = 1; i < 4; ++i) {
-    const float r = __fadd_rn(s, t[i]), v = __fsub_rn(r, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(r, v)), __fsub_rn(t[i], v)));
-    s = r;
+    s = two_sum(s, t[i], t[i]);
+    e = two_sum(e, t[i], t[i]);
+    e2 = __fadd_rn(e2, t[i]);
   }
-  if (!isfinite(s)) return ((double(t[0]) + double(t[1])) + double(t[2])) + double(t[3]);
-  return double(s) + double(e);
+  if (!isfinite(s)) return ((double(term(0)) + double(term(1))) + double(term(2))) + double(term(3));
+  return (double(s) + double(e)) + double(e2);
 }
 
 template <typename ST>

@@ -97,6 +97,17 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// Waits until a copy or an MMA in flight has landed, before shared memory or TMEM is
+// released.  Does not give up on an abort, nor at a short spin limit: the caller's limit
+// says how long the kernel waits for its work, and what is in flight then still lands.
+constexpr long long kDrainProbes = 1ll << 20;
+__device__ __forceinline__ void wait_drain(uint64_t* bar, uint32_t parity, long long limit) {
+  const uint32_t a = smem_u32(bar);
+  const long long n = limit > kDrainProbes ? limit : kDrainProbes;
+  for (long long i = 0; i < n; ++i)
+    if (mbar_test_cta(a, parity)) return;
+}
+
 // A position in a ring of mbarriers: the slot and the parity of its current use.
 // Counted, not divided: a 64-bit division by a run-time ring size in front of
 // every wait costs the issuing warps more than the waits themselves.

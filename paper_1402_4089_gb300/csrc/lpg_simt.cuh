@@ -398,8 +398,9 @@ __device__ __forceinline__ void lpg_body(const LpgArgs& A, const int cl) {
       if (lane < rv) bulk_g2s(xs + (size_t(slot) * BM + lane) * xpitch, src + size_t(lane) * A.p_pad, row_bytes, &full[slot]);
     }
     // Every copy must land before shared memory is released.
+    wait_drain(bbar, 0u, A.spin_limit);
     for (int64_t t = max(int64_t(0), T - NSTAGE); t < T; ++t)
-      (void)mbar_wait_cta(&full[t % NSTAGE], uint32_t((t / NSTAGE) & 1), A.spin_limit);
+      wait_drain(&full[t % NSTAGE], uint32_t((t / NSTAGE) & 1), A.spin_limit);
   } else if (logit) {
     // ---------------------------------------------------------------- logit group
     const int ga = lane / P, gc = lane % P;        // row group, phase

@@ -83,13 +83,6 @@ constexpr int kACols = 96;                   // TMEM columns of one A buffer: 3 
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxN = kSplitMaxN;
 constexpr int kHalfN = 32;                   // columns of a set of accumulators at most: five each, 2 A buffers + 2 sets = 512
-// Does not give up on the abort flag: a role sees its own copies or MMAs land
-// before shared memory or TMEM is released.
-__device__ __forceinline__ void wait_drain(uint64_t* bar, uint32_t parity, long long limit) {
-  const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < limit; ++i)
-    if (mbar_test_cta(a, parity)) return;
-}
 
 // D[tmem] (+)= A[tmem] B[smem], BF16 operands, FP32 accumulation.
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {

@@ -157,14 +157,6 @@ __device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, lon
   return false;
 }
 
-// Does not give up on the abort flag: a role sees its own copies or MMAs land before
-// shared memory or TMEM is released.
-__device__ __forceinline__ void wait_drain(uint64_t* bar, uint32_t parity, long long limit) {
-  const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < limit; ++i)
-    if (mbar_test_cta(a, parity)) return;
-}
-
 // Chunk c of row r of zx sits at chunk c ^ zx_swizzle(r, N): eight consecutive rows
 // then hold a class in eight different bank groups (N is a multiple of 16, so a row
 // starts at bank 0, or at bank 0 or 16 in turn).
@@ -209,7 +201,7 @@ struct TcShare {
 
 // One cluster's share of the fused pass for problem A.  `base` is the TMEM the
 // kernel allocated; nullptr: the body allocates what it needs.  `stop`: raised in
-// every CTA of the cluster if a wait ran out (only with `base`).
+// every CTA of the cluster if a wait ran out (nullptr: a word of the body's own).
 template <bool kFP8>
 __device__ __forceinline__ void tc_body(const TcArgs& A, const TcShare& W, const uint32_t* base, int* stop) {
   constexpr int kThreads = kFP8 ? kThreadsFp8 : kThreadsBf16;
@@ -250,6 +242,7 @@ __device__ __forceinline__ void tc_body(const TcArgs& A, const TcShare& W, const
   uint64_t* never = gdone + 3;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gdone + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gdone + 5);
+  if (!stop) stop = reinterpret_cast<int*>(gdone + 6);
   const size_t rbuf_bytes = size_t(NP / kBox) * kBoxBytes;
 
   if (tid == 0) {
@@ -272,6 +265,7 @@ __device__ __forceinline__ void tc_body(const TcArgs& A, const TcShare& W, const
     mbar_init(&drain[1], 1);
     mbar_init(never, 1);
     *abort_flag = 0;
+    *stop = 0;
     fence_mbar_init_cluster();
   }
   // R operand buffer and the local R rows start (and stay, past column C) zero.
@@ -752,13 +746,18 @@ __device__ __forceinline__ void tc_body(const TcArgs& A, const TcShare& W, const
     fence_after_sync();
     tmem_dealloc(tmem, A.tmem_cols);
   }
-  if (base && *abort_flag && tid < S) {
+  if (*abort_flag && tid < S) {
     const uint32_t a = smem_u32(stop);
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(S > 1 ? map_peer(a, uint32_t(tid)) : a), "r"(1) : "memory");
   }
   if (S > 1) cluster_sync_all();
-  if (base) {   // the next share lays out its own barriers here
-    if (S == 1) __syncthreads();
+  else __syncthreads();
+  if (*reinterpret_cast<volatile int*>(stop)) {
+    // Without an abort every push between CTAs has been waited for.  After one, some of
+    // those that the cluster issued before the barrier may be on their way: the shared
+    // memory and the barriers that they go to stay until they have landed.
+    __nanosleep(200000);
+  } else if (base) {   // the next share lays out its own barriers here
     for (int i = tid; i < 3 * nslots + 6 * kMaxDepth + kMaxAhead + 1 + 4; i += kThreads)
       asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bars + i)) : "memory");
   }

@@ -99,15 +99,6 @@ __device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity, lon
   return false;
 }
 
-// Bounded wait that does not give up on the abort flag: used where a role must
-// see its own bulk copies or MMAs complete before shared memory or TMEM is
-// released, also on the error path.
-__device__ __forceinline__ void wait_drain(uint64_t* bar, uint32_t parity, long long limit) {
-  const uint32_t a = smem_u32(bar);
-  for (long long i = 0; i < limit; ++i)
-    if (mbar_test_cta(a, parity)) return;
-}
-
 // Pass A's epilogue barrier over its T threads.
 template <int T>
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory"); }

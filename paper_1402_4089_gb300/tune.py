@@ -17,6 +17,11 @@ CUDA-core engine (FP32 / FP64 X), whose plans the library derives from the
 shape (one candidate each).  With engine 0 every engine the
 storage type allows is a candidate.  Tiles the library rejects for the shape
 are skipped.
+
+A small FP32 / FP64 problem, which the library by itself runs in one launch per call
+(engine 0, no tile), has no fused launches to time and loses that path with any explicit
+tile.  With engine 0 the fastest tile is therefore compared with it by the time of a
+leapfrog step, and the library's own choice is kept where it is faster.
 """
 import json
 import os
@@ -92,10 +97,42 @@ def time_tile(X, y, K, prior, prior_scale, x_storage, state, chains, engine, til
         h.close()
 
 
+def time_steps(X, y, K, prior, prior_scale, x_storage, state, chains, engine, tile, stream=None, reps=5,
+               layout="free"):
+    """Median time (us) of a leapfrog step of all `chains`, over trajectories of ten; with engine 0 and
+    no tile, None unless the library runs them in one launch."""
+    import torch
+    if not torch.cuda.is_available():
+        return None
+    steps = 10
+    h = hmc.create(X, y, K, prior, prior_scale, x_storage=x_storage, state=state, max_chains=chains, engine=engine,
+                   stream=stream, tile=tile, layout=layout)
+    try:
+        if not engine and not tile and not h.describe()["problems"][0].get("one_launch"):
+            return None
+        s = stream if stream is not None else torch.cuda.current_stream()
+        times = []
+        with torch.cuda.stream(s):
+            dev = torch.device("cuda", torch.cuda.current_device())
+            q = torch.zeros((chains, h.rows(), int(X.shape[1])), dtype=h.torch_dtype(), device=dev)
+            m, g = torch.zeros_like(q), torch.zeros_like(q)
+            for i in range(reps + 3):      # the ordinary path captures its launches in the first calls
+                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                e0.record(s)
+                h.leapfrog(q, m, steps, 1e-6, grad=g)
+                e1.record(s)
+                torch.cuda.synchronize()
+                if i >= 3:
+                    times.append(e0.elapsed_time(e1) * 1e3 / steps)
+        return float(np.median(times))
+    finally:
+        h.close()
+
+
 def autotune(X, y, K, prior="gaussian", prior_scale=1.0, x_storage="f32", state="f32", chains=1, engine=0,
              stream=None, reps=5, use_cache=True, verbose=False, layout="free"):
     """Fastest (engine, tile) for this problem: returns (engine, tile tuple for hmc.create, table of
-    measurements); (engine, None, table) when no explicit tile runs."""
+    measurements); (engine, None, table) when no explicit tile runs or the library's own choice is faster."""
     import torch
     n, p = int(X.shape[0]), int(X.shape[1])
     if engine:
@@ -107,7 +144,7 @@ def autotune(X, y, K, prior="gaussian", prior_scale=1.0, x_storage="f32", state=
     cache = _load() if use_cache else {}
     if key in cache:
         e = cache[key]
-        return int(e["engine"]), tuple(e["tile"]), e.get("table", [])
+        return int(e["engine"]), tuple(e["tile"]) if e["tile"] else None, e.get("table", [])
     table = []
     for eng in engines:
         cands = [(0, 0)] if eng in (3, 4) else [(S, ns) for S in (TC_S if eng == 2 else SIMT_S) for ns in RING]
@@ -126,9 +163,16 @@ def autotune(X, y, K, prior="gaussian", prior_scale=1.0, x_storage="f32", state=
         # No explicit tile runs for this shape: leave the choice to the library.
         return engine, None, table
     best = min(table, key=lambda r: r["us"])
-    tile = (best["S"], 0, 0, best["ring"])
+    chosen, tile = best["engine"], (best["S"], 0, 0, best["ring"])
+    if not engine and x_storage in ("f32", "f64"):
+        args = (X, y, K, prior, prior_scale, x_storage, state, chains)
+        kw = dict(stream=stream, reps=reps, layout=layout)
+        own = time_steps(*args, 0, None, **kw)
+        if own is not None and own < time_steps(*args, chosen, tile, **kw):
+            chosen, tile = 0, None
+            table.append(dict(engine=0, S=0, ring=0, us=round(own, 2), clusters=None, group_chains=chains, smem=None))
     if use_cache:
         cache = _load()
-        cache[key] = dict(engine=best["engine"], tile=list(tile), table=table)
+        cache[key] = dict(engine=chosen, tile=list(tile) if tile else None, table=table)
         _store(cache)
-    return best["engine"], tile, table
+    return chosen, tile, table

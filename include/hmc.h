@@ -86,7 +86,8 @@ typedef enum { HMC_F64 = 0, HMC_F32 = 1, HMC_BF16 = 2, HMC_FP8E4M3 = 3 } hmc_dty
 typedef struct {
   hmc_dtype x_storage;    /* storage type of X on the device (default HMC_F32)   */
   hmc_dtype state;        /* HMC_F64 or HMC_F32 (default HMC_F32)                */
-  int32_t max_chains;     /* largest `chains` any later call may pass (default 1) */
+  int32_t max_chains;     /* largest `chains` any later call may pass (default 1); the engine and its
+                             plan are chosen for calls with that many */
   int32_t engine;         /* 0 auto, 1 CUDA-core fused kernel, 2 tensor-core fused kernel (BF16 or
                              FP8 storage; MMA operands BF16, FP32 accumulation), 3 tensor-core
                              two-pass kernels (BF16 or FP8 storage, FP8 codes widened to BF16 in
@@ -322,7 +323,10 @@ const char* hmc_describe(hmc_handle h);
  * measured with CUDA events on the handle's stream around every fused launch
  * once enabled with hmc_set_timing(h, 1), or around every k-th one with
  * hmc_set_timing(h, k) for k > 1 (fewer events in a captured iteration);
- * enabling resets the totals: total milliseconds and timed launches since then.  hmc_sample replays a captured
+ * enabling resets the totals: total milliseconds and timed launches since then.
+ * While timing is on, a problem that runs in one launch ("one_launch" of
+ * hmc_describe) takes the ordinary launches, which have a fused kernel to time;
+ * their results differ in rounding.  hmc_sample replays a captured
  * graph per iteration without synchronising between replays; its events are
  * read after the last iteration, so a sampling call contributes the launches
  * of its last iteration.

@@ -1221,6 +1221,9 @@ hmc_status validate_opts(const hmc_opts* o) {
   return HMC_OK;
 }
 
+// Longest estimated launch of a small problem's trajectories.
+constexpr double kSmallLaunchUs = 20000.0;
+
 void build_description(hmc_ctx* h) {
   const int e0 = h->probs.empty() ? 1 : h->probs[0].engine;
   std::string s = "{\"engine\": \"" + std::string(e0 == 1 ? "simt" : e0 == 2 ? "tcgen05" : e0 == 3 ? "tcgen05_2pass" : "simt_2pass") +
@@ -1250,7 +1253,8 @@ void build_description(hmc_ctx* h) {
       s.insert(s.size() - 1, buf);   // inside this problem's object
     }
     if (P.small.S) {
-      std::snprintf(buf, sizeof(buf), ", \"one_launch\": {\"cluster\": %d, \"smem\": %zu}", P.small.S, P.small.smem);
+      std::snprintf(buf, sizeof(buf), ", \"one_launch\": {\"cluster\": %d, \"smem\": %zu, \"launch_steps\": %lld}", P.small.S,
+                    P.small.smem, (long long)(kSmallLaunchUs / P.small.us));
       s.insert(s.size() - 1, buf);
     }
     if (P.engine == 4) {
@@ -1429,14 +1433,10 @@ hmc_status check_chains(hmc_ctx* h, int chains) {
   return HMC_OK;
 }
 
-// log K and gradient at the state in `S` for every problem.
 // Enqueue `body` (work on h->stream) directly, or through the call graph of
 // `slot` when `cacheable` (device buffers only, no timing events, no pending
 // fault injection): the second identical call in a row is captured on the
 // private stream and launched as a graph, later ones replay it.
-// Longest estimated launch of a small problem's trajectories.
-constexpr double kSmallLaunchUs = 20000.0;
-
 template <typename F>
 hmc_status run_cached(hmc_ctx* h, int slot, std::vector<uint64_t> key, bool cacheable, F body) {
   hmc_ctx::CallGraph& g = h->cg[slot];
@@ -1647,10 +1647,10 @@ hmc_status hmc_logpost_grad(hmc_handle h, const void* beta, int32_t chains, doub
     small_user(a, *P, bd, nullptr, nullptr, gd, static_cast<double*>(ld));
     HMC_CUDA(small_launch(h->xt, P->small, a, chains, h->stream));
   } else {
-  HMC_TRY(run_cached(h, 0, {uint64_t(chains), key_of(bd), key_of(gd), key_of(ld)}, cacheable, [&]() -> hmc_status {
-    HMC_TRY(pack_all(h, bd, chains, false, &StateSet::beta));
-    return eval_state(h, false, chains, gd, static_cast<double*>(ld));
-  }));
+    HMC_TRY(run_cached(h, 0, {uint64_t(chains), key_of(bd), key_of(gd), key_of(ld)}, cacheable, [&]() -> hmc_status {
+      HMC_TRY(pack_all(h, bd, chains, false, &StateSet::beta));
+      return eval_state(h, false, chains, gd, static_cast<double*>(ld));
+    }));
   }
   if (gh) HMC_CUDA(cudaMemcpyAsync(grad, gd, bytes, cudaMemcpyDeviceToHost, h->stream));
   if (lh)
@@ -1691,38 +1691,38 @@ hmc_status hmc_leapfrog(hmc_handle h, void* beta, void* eta, void* grad, double*
     a.eps = eps;
     HMC_CUDA(small_launch(h->xt, sp->small, a, chains, h->stream));
   } else {
-  HMC_TRY(run_cached(h, 1, {uint64_t(chains), uint64_t(L), eps_bits, key_of(bd), key_of(ed), key_of(gd), key_of(ld)},
-                     cacheable, [&]() -> hmc_status {
-    HMC_TRY(pack_all(h, bd, chains, false, &StateSet::beta));
-    HMC_TRY(pack_all(h, ed, chains, false, &StateSet::eta));
-    if (gd) {
-      HMC_TRY(pack_all(h, gd, chains, false, &StateSet::grad));
-    }
-    if (!gd || L == 0) HMC_TRY(eval_state(h, false, chains));
-    if (L > 0) {
-      for (size_t b = 0; b < h->probs.size(); ++b) {
-        UpdateArgs u = make_update(h, h->probs[b], h->probs[b].us, 1, chains, eps, int(b));
-        HMC_CUDA(launch_leap_start(h->st, u, h->stream));
+    HMC_TRY(run_cached(h, 1, {uint64_t(chains), uint64_t(L), eps_bits, key_of(bd), key_of(ed), key_of(gd), key_of(ld)},
+                       cacheable, [&]() -> hmc_status {
+      HMC_TRY(pack_all(h, bd, chains, false, &StateSet::beta));
+      HMC_TRY(pack_all(h, ed, chains, false, &StateSet::eta));
+      if (gd) {
+        HMC_TRY(pack_all(h, gd, chains, false, &StateSet::grad));
       }
-      for (int l = 1; l <= L; ++l) {
-        HMC_TRY(run_lpg_all(h, false, chains, h->stream));
-        const int mode = (l < L) ? (UPD_ETA_FULL | UPD_BETA) : (UPD_ETA_HALF | UPD_SCALARS);
-        if (h->u_table) {
-          HMC_CUDA(launch_reduce_update_batched(h->st, make_batch(h, false, chains, eps), mode, h->stream));
-          continue;
-        }
+      if (!gd || L == 0) HMC_TRY(eval_state(h, false, chains));
+      if (L > 0) {
         for (size_t b = 0; b < h->probs.size(); ++b) {
           UpdateArgs u = make_update(h, h->probs[b], h->probs[b].us, 1, chains, eps, int(b));
-          HMC_CUDA(launch_reduce_update(h->st, u, mode, h->stream));
+          HMC_CUDA(launch_leap_start(h->st, u, h->stream));
+        }
+        for (int l = 1; l <= L; ++l) {
+          HMC_TRY(run_lpg_all(h, false, chains, h->stream));
+          const int mode = (l < L) ? (UPD_ETA_FULL | UPD_BETA) : (UPD_ETA_HALF | UPD_SCALARS);
+          if (h->u_table) {
+            HMC_CUDA(launch_reduce_update_batched(h->st, make_batch(h, false, chains, eps), mode, h->stream));
+            continue;
+          }
+          for (size_t b = 0; b < h->probs.size(); ++b) {
+            UpdateArgs u = make_update(h, h->probs[b], h->probs[b].us, 1, chains, eps, int(b));
+            HMC_CUDA(launch_reduce_update(h->st, u, mode, h->stream));
+          }
         }
       }
-    }
-    HMC_TRY(unpack_all(h, bd, chains, false, &StateSet::beta));
-    HMC_TRY(unpack_all(h, ed, chains, false, &StateSet::eta));
-    if (gd) HMC_TRY(unpack_all(h, gd, chains, false, &StateSet::grad));
-    if (ld) HMC_TRY(copy_logk(h, static_cast<double*>(ld), chains, 1));
-    return HMC_OK;
-  }));
+      HMC_TRY(unpack_all(h, bd, chains, false, &StateSet::beta));
+      HMC_TRY(unpack_all(h, ed, chains, false, &StateSet::eta));
+      if (gd) HMC_TRY(unpack_all(h, gd, chains, false, &StateSet::grad));
+      if (ld) HMC_TRY(copy_logk(h, static_cast<double*>(ld), chains, 1));
+      return HMC_OK;
+    }));
   }
   if (bh) HMC_CUDA(cudaMemcpyAsync(beta, bd, bytes, cudaMemcpyDeviceToHost, h->stream));
   if (eh) HMC_CUDA(cudaMemcpyAsync(eta, ed, bytes, cudaMemcpyDeviceToHost, h->stream));

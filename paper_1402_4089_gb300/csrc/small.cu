@@ -4,7 +4,7 @@
 //
 // A small gradient is bound by launches and by the latency of passing partial sums
 // through global memory: n=1000 p=50 K=3 in FP64 took 20.6 us a leapfrog step as two
-// launches and takes 10.2 here (a chain of FP64 operations, about 100 clocks each, most
+// launches and takes 10.6 here (a chain of FP64 operations, about 100 clocks each, most
 // of it: dots 5500, softmax 4200, X^T R 7600 of 20700 clocks), n=100 p=10 K=2 in FP32
 // 10.2 and 2.3.
 // Here a cluster of S CTAs keeps X in shared memory (rows split over the CTAs), every
